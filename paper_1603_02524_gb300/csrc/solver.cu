@@ -402,21 +402,27 @@ void attach_split(FdmFamily<T>& fam, const LevelDims& dm, const AxisTables* cons
     ax.SF = upload_frag(own, sf);
     ax.WF = upload_frag(own, wf);
   }
-  // offset of every node of every position: element-major, wrapped on periodic axes
+  // offset of every node of every position: element-major, wrapped on periodic axes; on an axis
+  // of stacked copies (bpos positions each) only the nodes of the position's own copy: beyond its
+  // walls the tables are zero, but the digit-split kernel scales a patch by its largest value
   const long long nodes_el = (long long)dm.NP * dm.NP * dm.NPz;
   const long long es[3] = {nodes_el, nodes_el * dm.ne[0], nodes_el * dm.ne[0] * dm.ne[1]};
   const long long ns[3] = {1, dm.NP, (long long)dm.NP * dm.NP};
   for (int q = 0; q < 3; ++q) {
     FdmAxis<T>& ax = fam.ax[q];
     const int npp = ax.phys == 2 ? dm.NPz : dm.NP;
+    const int own_nodes = ax.bpos ? ax.N / (ax.count / ax.bpos) : ax.N;
     std::vector<long long> off((size_t)ax.count * ax.n);
-    for (int p = 0; p < ax.count; ++p)
+    for (int p = 0; p < ax.count; ++p) {
+      const int lo = ax.bpos ? p / ax.bpos * own_nodes : 0;
       for (int a = 0; a < ax.n; ++a) {
         int G = patch_start(ax, p, npp) + a;
         if (ax.periodic) G = ((G % ax.N) + ax.N) % ax.N;
-        off[(size_t)p * ax.n + a] =
-            (G < 0 || G >= ax.N) ? kInvalidOffset : (long long)(G / npp) * es[ax.phys] + (G % npp) * ns[ax.phys];
+        off[(size_t)p * ax.n + a] = (G < lo || G >= lo + own_nodes)
+                                        ? kInvalidOffset
+                                        : (long long)(G / npp) * es[ax.phys] + (G % npp) * ns[ax.phys];
       }
+    }
     long long* d = dev_alloc<long long>(own, off.size());
     PMG_CUDA(cudaMemcpy(d, off.data(), off.size() * sizeof(long long), cudaMemcpyHostToDevice));
     ax.goff = d;
