@@ -662,14 +662,14 @@ struct PatchRows {
       }
     }
   }
-  // u += get(row NA + a) on the rows' valid entries
+  // u += get(row NA + a, row) on the rows' valid entries
   template <int NR, typename T, typename Get>
   __device__ __forceinline__ void scatter(T* __restrict__ u, const long long* rowoff, Get&& get) const {
     if (offa < 0) return;
 #pragma unroll 4
     for (int rr = row; rr < NR; rr += step) {
       const long long o = offa + rowoff[rr];
-      if (o >= 0) atomicAdd(u + o, get(rr * NA + a));
+      if (o >= 0) atomicAdd(u + o, get(rr * NA + a, rr));
     }
   }
 };

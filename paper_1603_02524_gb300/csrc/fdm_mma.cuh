@@ -272,7 +272,7 @@ fdm_kernel_mma(FdmFamily<float> fam, const float* __restrict__ r, float* __restr
   __syncthreads();
   mma_pass<NA, false>(fold[0], Fb[0], buf, NB * NC, 1, base_a, plain);
   __syncthreads();
-  rows.template scatter<NB * NC>(u, rowoff, [&](int t) { return buf[t]; });
+  rows.template scatter<NB * NC>(u, rowoff, [&](int t, int) { return buf[t]; });
 }
 
 template <int NA, int NB, int NC>

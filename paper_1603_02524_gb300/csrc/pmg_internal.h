@@ -144,6 +144,7 @@ struct FdmAxis {
   // split.cuh, with their two exponents in fexp; fp32: bf16 terms, fdm_mma.cuh)
   const int* fid;
   const int* fexp;
+  const int* wexp;         // FP64: exponent of each of the n outputs of a distinct W table
   const long long* goff;   // [count][n] offset contribution of each node (negative: outside)
   const uint4* SF;
   const uint4* WF;

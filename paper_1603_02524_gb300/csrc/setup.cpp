@@ -788,6 +788,27 @@ SplitBlocks patch_blocks(const double* M, int n, bool folded, bool backward) {
   return B;
 }
 
+// Each output node of a backward patch table scaled by a power of two of its own (two mirrored
+// nodes alike): the weights of the additive update make the rows of the outer nodes up to 1e-6
+// of the others, which would lose that much of their precision.
+void scale_patch_outputs(SplitBlocks& B, int n, bool folded, int* rexp) {
+  const int nt = (n + 15) / 16;
+  for (int o = 0; o < n; ++o) {
+    const int row = folded ? std::min(o, n - 1 - o) : o & 15;
+    const int b0 = folded ? 0 : (o >> 4) * nt, nb = folded ? 2 : nt;
+    if (folded && row != o) {
+      rexp[o] = rexp[row];
+      continue;
+    }
+    double s = 0.0;
+    for (int b = b0; b < b0 + nb; ++b)
+      for (int k = 0; k < 16; ++k) s += std::fabs(B.at(b, k, row));
+    std::frexp(s, rexp + o);                               // 0 for an empty row
+    for (int b = b0; b < b0 + nb; ++b)
+      for (int k = 0; k < 16; ++k) B.at(b, k, row) = std::ldexp(B.at(b, k, row), -rexp[o]);
+  }
+}
+
 // Exponent shift of the neighbour derivatives: sum_k |D_{P,k}| <= 2^kd.
 int apply_deriv_shift(const Axis1DHost& a) {
   double s = 0.0;

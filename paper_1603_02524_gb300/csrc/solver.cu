@@ -367,7 +367,7 @@ void attach_split(FdmFamily<T>& fam, const LevelDims& dm, const AxisTables* cons
     if (q == 0)
       for (double& x : t.W) x *= omega;
     const size_t nn = (size_t)n * n, len = (size_t)split_blocks(n) * (fp64 ? kSplitDigits : kBf16Terms) * 32 * 4;
-    std::vector<int> fid(t.count), reps, expo;
+    std::vector<int> fid(t.count), reps, expo, wexp;
     std::vector<uint32_t> sf, wf;
     for (int p = 0; p < t.count; ++p) {
       int f = -1;
@@ -384,8 +384,10 @@ void attach_split(FdmFamily<T>& fam, const LevelDims& dm, const AxisTables* cons
         wf.resize(wf.size() + len);
         expo.resize(expo.size() + 2);
         const SplitBlocks S = patch_blocks(&t.S[p * nn], n, t.sym[p] != 0, false);
-        const SplitBlocks W = patch_blocks(&t.W[p * nn], n, t.sym[p] != 0, true);
+        SplitBlocks W = patch_blocks(&t.W[p * nn], n, t.sym[p] != 0, true);
         if (fp64) {
+          wexp.resize(wexp.size() + n);
+          scale_patch_outputs(W, n, t.sym[p] != 0, &wexp[(size_t)f * n]);
           split_fragments(S, expo[2 * f], ok, &sf[f * len]);
           split_fragments(W, expo[2 * f + 1], ok, &wf[f * len]);
         } else {
@@ -398,7 +400,10 @@ void attach_split(FdmFamily<T>& fam, const LevelDims& dm, const AxisTables* cons
     }
     FdmAxis<T>& ax = fam.ax[q];
     ax.fid = dev_upload_int(own, fid);
-    if (fp64) ax.fexp = dev_upload_int(own, expo);
+    if (fp64) {
+      ax.fexp = dev_upload_int(own, expo);
+      ax.wexp = dev_upload_int(own, wexp);
+    }
     ax.SF = upload_frag(own, sf);
     ax.WF = upload_frag(own, wf);
   }

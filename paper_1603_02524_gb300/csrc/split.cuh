@@ -5,16 +5,17 @@
 //
 // A table entry and a line value are fixed-point integers cut into six balanced
 // base-1024 digits, which fp16 holds exactly.  The products of digits i and j with
-// i + j = w are summed by fp16 MMAs into one fp32 accumulator per weight w = 0..5.
-// Every such sum is an integer below 2^24 (split_fragments checks the bound for each
-// table), so the accumulators are exact and the six of them, added as 64-bit
-// integers, give the product to about 2^-58 of (largest value) x (largest entry):
-// the terms w >= 6 that are left out are below that.
+// i + j = w are summed by fp16 MMAs into one fp32 accumulator per weight w = 0..6.
+// The sums w <= 3 are integers below 2^24 (split_fragments checks the bound for each
+// table), so these accumulators are exact, and the rounding of the others does not count;
+// added as 64-bit integers they give the product to about 2^-60 of (largest value) x
+// (largest entry).  Without the weight 6 the error of P = 16 sweeps against 64 bits was a third above
+// that of the plain FP64 kernel (EA 1.02e-14 against 7.9e-15); the terms w >= 7 are below 2^-60.
 //
 // Scaling: B = M 2^(59 - e), where sum_k |M_k| <= 2^e for every output of the table (one e
 // per table; a backward even-odd table counts both blocks of a node); X = x 2^-ex with
 // |X| < 2^60.  B = sum_j b_j 2^(50 - 10 j), X = sum_i x_i 2^(52 - 10 i), hence
-// sum M x = T 2^(e + 2 + ex) with T = sum_w acc_w 2^(41 - 10 w), |T| <= 2^58.
+// sum M x = T 2^(e + 2 - g + ex) with T = sum_w acc_w 2^(41 + g - 10 w), |T| <= 2^(58 + g).
 #pragma once
 
 #include <cstdint>
@@ -25,6 +26,7 @@
 namespace pmg {
 
 constexpr int kSplitDigits = 6;
+constexpr int kSplitWeights = 7;
 
 // blocks of 16 x 16 table entries per table: one up to 16 nodes; above, those of a general
 // table (up to 32 nodes an even-odd folded one takes the first two)
@@ -51,6 +53,9 @@ void bf16_fragments(const SplitBlocks& B, uint32_t* frag);
 // the same fragments for the table as the second MMA operand (n > 32, the slab kernel's c-lines)
 void bf16_fragments_b(const SplitBlocks& B, uint32_t* frag);
 SplitBlocks patch_blocks(const double* M, int n, bool folded, bool backward);
+// scales every output of a backward patch table to entries that sum to about 1; rexp[n]: the
+// exponents taken out
+void scale_patch_outputs(SplitBlocks& B, int n, bool folded, int* rexp);
 // 1-D operator of element m of an axis with its neighbour terms as further inputs (see
 // setup.cpp); kd: the derivative inputs come times 2^-kd.  folded: even-odd form.  rexp[NP]:
 // exponent of each output.
@@ -119,8 +124,19 @@ __device__ __forceinline__ void split_mma(float (&acc)[NW][4], const uint4 (&A)[
     }
 }
 
-// T = sum_w acc_w 2^(41 - 10 w), the last two accumulators merged in fp32; |acc_0| < 2^18
-// and |acc_1| < 2^23 by the row-sum scaling, so the first two merge in 32 bits
+// T = sum_w acc_w 2^(42 - 10 w), the last three accumulators merged in fp32; |acc_0| < 2^18
+// and |acc_1| < 2^23 by the row-sum scaling, so the first two merge in 32 bits.  |T| <= 2^59,
+// so the next pass's normalisation never shifts to the right.
+__device__ __forceinline__ long long split_join_patch(const float (&acc)[kSplitWeights][4], int r) {
+  const int i0 = __float2int_rn(acc[0][r]), i1 = __float2int_rn(acc[1][r]), i2 = __float2int_rn(acc[2][r]),
+            i3 = __float2int_rn(acc[3][r]),
+            i4 = __float2int_rn(__fmaf_rn(acc[4][r], 4.0f, __fmaf_rn(acc[6][r], 0x1p-18f, acc[5][r] * 0x1p-8f)));
+  long long T = (long long)i3 * 4096 + i4;
+  T += (long long)i2 * 4194304;
+  return T + (long long)((unsigned long long)(unsigned)(i0 * 1024 + i1) << 32);
+}
+
+// T = sum_w acc_w 2^(41 - 10 w) of six weights
 __device__ __forceinline__ long long split_join(const float (&acc)[kSplitDigits][4], int r) {
   const int i0 = __float2int_rn(acc[0][r]), i1 = __float2int_rn(acc[1][r] + acc[1][r]),
             i2 = __float2int_rn(acc[2][r]), i3 = __float2int_rn(acc[3][r]),
@@ -131,10 +147,8 @@ __device__ __forceinline__ long long split_join(const float (&acc)[kSplitDigits]
 }
 
 // The operator apply subtracts large terms (its results are far below row sum x largest
-// value), so it also takes the products of weight 6 and keeps three more bits:
-// T = sum_w acc_w 2^(44 - 10 w), |T| <= 2^61.
-constexpr int kApplyWeights = 7;
-__device__ __forceinline__ long long split_join(const float (&acc)[kApplyWeights][4], int r) {
+// value), so it keeps more bits: T = sum_w acc_w 2^(44 - 10 w), |T| <= 2^61.
+__device__ __forceinline__ long long split_join(const float (&acc)[kSplitWeights][4], int r) {
   const int i0 = __float2int_rn(acc[0][r]), i1 = __float2int_rn(acc[1][r]), i2 = __float2int_rn(acc[2][r]),
             i3 = __float2int_rn(acc[3][r]),
             i4 = __float2int_rn(__fmaf_rn(acc[4][r], 16.0f, __fmaf_rn(acc[6][r], 0x1p-16f, acc[5][r] * 0x1p-6f)));
@@ -168,6 +182,11 @@ __device__ __forceinline__ double scaled_double(unsigned long long a, bool neg, 
 // pipe, about 75 times one of these); the result must lie in the normal range
 __device__ __forceinline__ double fixed_double(long long T, int k) {
   return scaled_double((unsigned long long)(T < 0 ? -T : T), T < 0, k);
+}
+// the same for any k
+static __device__ __noinline__ double any_double(long long T, int k) { return scalbn((double)T, k); }
+__device__ __forceinline__ double fixed_double_any(long long T, int k) {
+  return (unsigned)(k + 1000) < 1900u ? fixed_double(T, k) : any_double(T, k);
 }
 
 #endif  // __CUDACC__
