@@ -7,7 +7,7 @@ import pytest
 
 import synthetic as syn
 from oracle import dg, schwarz
-from tests.helpers import e2g, elem_shape, from_dev, to_dev
+from tests.helpers import e2g, elem_shape, from_dev, g2e, to_dev
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -34,3 +34,80 @@ def test_sweep_precision_under_small_weights(P, overlap, fam):
     got = np.moveaxis(e2g(from_dev(out, shape), 3), 2 - fam, 0)
     for k in range(2 * P + 1):
         assert np.abs(got[k] - ref[k]).max() <= 1e-11 * np.abs(ref[k]).max()
+
+
+GRID = [[0.25] * 4, [0.5] * 2, [0.3, 0.7]]
+
+
+@pytest.mark.parametrize("big", [1e12, 1e30, -1e250])
+@pytest.mark.parametrize("P", [4, 8, 16])
+def test_apply_off_the_lines_of_a_large_value(P, big):
+    """A u depends on the lines through a node: one large value changes nothing elsewhere."""
+    from paper_1603_02524_gb300 import Grid, Hierarchy
+    h = Hierarchy(Grid(3, P, [4, 2, 2], GRID, periodic=False))
+    shape = elem_shape(3, (4, 2, 2), P)
+    u = syn.rng(140).uniform(-1, 1, size=shape)
+    a, b = (torch.zeros(u.size, dtype=torch.float64, device="cuda") for _ in range(2))
+    h.apply(h.L, to_dev(u), a)
+    u[0, 0, 1, 1, 2, 2] = big
+    h.apply(h.L, to_dev(u), b)
+    hit = np.zeros(shape, dtype=bool)
+    hit[0, 0, :3, 1, 2, :] = hit[0, 0, 1, 1, :, 2] = hit[0, 0, 1, :, 2, 2] = True
+    hit[0, 1, 1, 1, :, 2] = hit[1, 0, 1, :, 2, 2] = True
+    got, ref = from_dev(b, shape), from_dev(a, shape)
+    assert np.abs(got[~hit] - ref[~hit]).max() <= 1e-13 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("small", [1e-6, 1e-15, 1e-290])
+@pytest.mark.parametrize("P", [4, 8, 16])
+def test_apply_at_small_edges(P, small):
+    """Values far smaller on two faces of every element (as next to a Dirichlet wall): the edge
+    between them depends on these alone and keeps the relative accuracy of the apply."""
+    from paper_1603_02524_gb300 import Grid, Hierarchy
+    h = Hierarchy(Grid(3, P, [4, 2, 2], GRID, periodic=False))
+    shape = elem_shape(3, (4, 2, 2), P)
+    u = syn.rng(141).uniform(-1, 1, size=shape)
+    u[..., 0, :] *= small
+    u[..., 0] *= small
+    u[..., 0, 0] /= small
+    out = torch.zeros(u.size, dtype=torch.float64, device="cuda")
+    h.apply(h.L, to_dev(u), out)
+    v = u.copy()                                           # the rest zero: the edge's result is the same
+    v[..., 1:, 1:] = 0.0
+    v /= small
+    ref = g2e(dg.Discretisation(3, P, GRID, False, 0.0, 1.0).apply(e2g(v, 3)), (4, 2, 2), P)[..., 0, 0]
+    got = from_dev(out, shape)[..., 0, 0] / small
+    assert np.abs(got - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("P", [4, 8, 16])
+def test_apply_of_a_localized_vector(P):
+    """Zero but for one element: the other elements' results are exact zeros, and they take no
+    longer than full ones (twice the time is the bound)."""
+    from paper_1603_02524_gb300 import Grid, Hierarchy
+    ne = (8, 8, 8)
+    sp = [[1 / n] * n for n in ne]
+    h = Hierarchy(Grid(3, P, ne, sp, periodic=False))
+    shape = elem_shape(3, ne, P)
+    u = np.zeros(shape)
+    u[4, 3, 2] = syn.rng(142).uniform(-1, 1, size=shape[3:])
+    full = torch.rand(u.size, dtype=torch.float64, device="cuda")
+    loc, out = to_dev(u), torch.empty_like(full)
+    h.apply(h.L, loc, out)
+    got = from_dev(out, shape)
+    near = np.zeros(shape[:3], dtype=bool)
+    near[4, 3, 1:4] = near[4, 2:5, 2] = near[3:6, 3, 2] = True
+    assert (got[~near] == 0.0).all() and (got[near] != 0.0).any()
+
+    def ms(x):
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                h.apply(h.L, x, out)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+    assert ms(loc) <= 2.0 * ms(full)
