@@ -637,23 +637,24 @@ void apply_rowform(const ApplyAxisHost& t, int NP, int W, std::vector<double>& L
   }
 }
 
-// fp16 bits of an integer |v| <= 1024 (exact)
+// fp16 bits of an integer |v| <= 2048 (exact)
 static uint32_t half_bits(int v) {
   if (v == 0) return 0;
   const uint32_t sign = v < 0 ? 0x8000u : 0u;
   uint32_t a = (uint32_t)(v < 0 ? -v : v);
   int e = 0;
   while ((a >> e) > 1) ++e;
-  return sign | (uint32_t)(e + 15) << 10 | ((a << (10 - e)) & 0x3ffu);
+  return sign | (uint32_t)(e + 15) << 10 | ((e > 10 ? a >> (e - 10) : a << (10 - e)) & 0x3ffu);
 }
 
 // Digit fragments of one table in the lane order of the m16n8k16 A operand: rows =
 // outputs, and lane t's K positions 2t, 2t + 1, 2t + 8, 2t + 9 hold inputs t, t + 4, t + 8,
-// t + 12 of a block.  expo: sum_k |entry| <= 2^expo for every output.  ok: with line digits
+// t + 12 of a block.  expo: sum_k |entry| <= 2^expo for every output; more_bits (up to 2): those
+// the table keeps below the 59 (its first digits grow to 2048).  ok: with line digits
 // of at most 512 (256 for the first), the accumulators of the weights 0..3 stay within 2^24
 // (and within the 32-bit merge of the first two), so they are exact; the unit of the last
 // two is below 2^-57 of the result's scale, where rounding does not count.
-void split_fragments(const SplitBlocks& B, int& expo, bool& ok, uint32_t* frag) {
+void split_fragments(const SplitBlocks& B, int& expo, bool& ok, uint32_t* frag, int more_bits) {
   const int D = kSplitDigits, nb = B.nblk;
   const int nacc = B.chain ? nb / 2 : nb;                  // accumulator sets
   double big = 0.0;
@@ -666,7 +667,7 @@ void split_fragments(const SplitBlocks& B, int& expo, bool& ok, uint32_t* frag) 
       big = std::max(big, s);
     }
   std::frexp(big * (1.0 + 1e-12), &expo);                  // big < 2^expo
-  const double scale = std::ldexp(1.0, 59 - expo);         // a power of two: exact
+  const double scale = std::ldexp(1.0, 59 + more_bits - expo);   // a power of two: exact
   std::vector<int> dig((size_t)nb * D * 256);              // [block][digit][row][k]
   std::vector<double> sums((size_t)D * nacc * 16, 0.0);    // [digit][accumulator set][row]
   unsigned long long bias = 0;
@@ -674,9 +675,10 @@ void split_fragments(const SplitBlocks& B, int& expo, bool& ok, uint32_t* frag) 
   for (int b = 0; b < nb; ++b)
     for (int row = 0; row < 16; ++row)
       for (int k = 0; k < 16; ++k) {
-        const unsigned long long Y = (unsigned long long)std::llround(B.at(b, k, row) * scale) + bias;
+        const long long Y = std::llround(B.at(b, k, row) * scale) + (long long)bias;
         for (int j = 0; j < D; ++j) {
-          const int d = (int)((Y >> (10 * (D - 1 - j))) & (j == 0 ? 0x3fffull : 0x3ffull)) - 512;
+          const long long q = Y >> (10 * (D - 1 - j));
+          const int d = (int)(j == 0 ? q : q & 0x3ff) - 512;
           dig[(((size_t)b * D + j) * 16 + row) * 16 + k] = d;
           sums[((size_t)j * nacc + (B.chain ? b / 2 : b)) * 16 + row] += std::abs(d);
         }
@@ -685,7 +687,7 @@ void split_fragments(const SplitBlocks& B, int& expo, bool& ok, uint32_t* frag) 
     for (int w = 0; w < 4; ++w) {
       double t = 0.0;
       for (int j = 0; j <= w; ++j) t += (w - j == 0 ? 256.0 : 512.0) * sums[(size_t)j * nacc * 16 + o];
-      if (t > (w == 0 ? 262144.0 : w == 1 ? 8388608.0 : 16777216.0)) ok = false;
+      if (t > (w == 0 ? 1048576.0 : w == 1 ? 8388608.0 : 16777216.0)) ok = false;
     }
   for (int b = 0; b < nb; ++b)
     for (int j = 0; j < D; ++j)

@@ -203,7 +203,7 @@ void attach_split_apply(Hier& h, int l, SplitApply& sp, std::vector<void*>& own)
         reps.push_back(B);
         frag.resize(frag.size() + len);
         int e = 0;
-        split_fragments(B, e, ok, &frag[f * len]);
+        split_fragments(B, e, ok, &frag[f * len], kApplyBits);
         info.push_back(folded ? 1 : 0);
         for (int o = 0; o < NP; ++o) info.push_back(e + rexp[o]);
         rexps.insert(rexps.end(), rexp.begin(), rexp.end());

@@ -12,10 +12,11 @@
 // (largest entry).  Without the weight 6 the error of P = 16 sweeps against 64 bits was a third above
 // that of the plain FP64 kernel (EA 1.02e-14 against 7.9e-15); the terms w >= 7 are below 2^-60.
 //
-// Scaling: B = M 2^(59 - e), where sum_k |M_k| <= 2^e for every output of the table (one e
-// per table; a backward even-odd table counts both blocks of a node); X = x 2^-ex with
-// |X| < 2^60.  B = sum_j b_j 2^(50 - 10 j), X = sum_i x_i 2^(52 - 10 i), hence
-// sum M x = T 2^(e + 2 - g + ex) with T = sum_w acc_w 2^(41 + g - 10 w), |T| <= 2^(58 + g).
+// Scaling: B = M 2^(59 + t - e), where sum_k |M_k| <= 2^e for every output of the table (one e
+// per table; a backward even-odd table counts both blocks of a node); t = 0, or 2 in the
+// operator's tables (kApplyBits); X = x 2^-ex with |X| < 2^60.  B = sum_j b_j 2^(50 - 10 j),
+// X = sum_i x_i 2^(52 - 10 i), hence sum M x = T 2^(e + 2 - g - t + ex) with
+// T = sum_w acc_w 2^(41 + g - 10 w), |T| <= 2^(58 + g + t).
 #pragma once
 
 #include <cstdint>
@@ -46,7 +47,8 @@ struct SplitBlocks {
   double& at(int b, int k, int o) { return v[((size_t)b * 16 + k) * 16 + o]; }
   double at(int b, int k, int o) const { return v[((size_t)b * 16 + k) * 16 + o]; }
 };
-void split_fragments(const SplitBlocks& B, int& expo, bool& ok, uint32_t* frag);
+constexpr int kApplyBits = 2;
+void split_fragments(const SplitBlocks& B, int& expo, bool& ok, uint32_t* frag, int more_bits = 0);
 // the same blocks as bf16 terms (fdm_mma.cuh), each entry the sum of three
 constexpr int kBf16Terms = 3;
 void bf16_fragments(const SplitBlocks& B, uint32_t* frag);
@@ -124,10 +126,10 @@ __device__ __forceinline__ void split_mma(float (&acc)[NW][4], const uint4 (&A)[
     }
 }
 
-// T = sum_w acc_w 2^(42 - 10 w), the last three accumulators merged in fp32; |acc_0| < 2^18
-// and |acc_1| < 2^23 by the row-sum scaling, so the first two merge in 32 bits.  |T| <= 2^59,
-// so the next pass's normalisation never shifts to the right.
-__device__ __forceinline__ long long split_join_patch(const float (&acc)[kSplitWeights][4], int r) {
+// T = sum_w acc_w 2^(42 - 10 w), the last three accumulators merged in fp32; |acc_0| < 2^20
+// and |acc_1| < 2^23 by the row-sum scaling, so the first two merge in 32 bits.  |T| <= 2^59 (2^61
+// with kApplyBits), so the normalisation of the next pass of a patch never shifts to the right.
+__device__ __forceinline__ long long split_join(const float (&acc)[kSplitWeights][4], int r) {
   const int i0 = __float2int_rn(acc[0][r]), i1 = __float2int_rn(acc[1][r]), i2 = __float2int_rn(acc[2][r]),
             i3 = __float2int_rn(acc[3][r]),
             i4 = __float2int_rn(__fmaf_rn(acc[4][r], 4.0f, __fmaf_rn(acc[6][r], 0x1p-18f, acc[5][r] * 0x1p-8f)));
@@ -146,27 +148,18 @@ __device__ __forceinline__ long long split_join(const float (&acc)[kSplitDigits]
   return T + (long long)(i0 * 2048 + i1) * 1073741824;
 }
 
-// The operator apply subtracts large terms (its results are far below row sum x largest
-// value), so it keeps more bits: T = sum_w acc_w 2^(44 - 10 w), |T| <= 2^61.
-__device__ __forceinline__ long long split_join(const float (&acc)[kSplitWeights][4], int r) {
-  const int i0 = __float2int_rn(acc[0][r]), i1 = __float2int_rn(acc[1][r]), i2 = __float2int_rn(acc[2][r]),
-            i3 = __float2int_rn(acc[3][r]),
-            i4 = __float2int_rn(__fmaf_rn(acc[4][r], 16.0f, __fmaf_rn(acc[6][r], 0x1p-16f, acc[5][r] * 0x1p-6f)));
-  long long T = (long long)i3 * 16384 + i4;
-  T += (long long)i2 * 16777216;
-  return T + (long long)(i0 * 1024 + i1) * 17179869184;
-}
-
-// x 2^(1081 - E) truncated, for the bits of a finite double below 2^(E - 1022), E >= 1
-// the biased exponent of the largest: |result| < 2^59
+// x 2^(1075 + UP - E) rounded down, for the bits of a finite double below 2^(E - 1022), E >= 1
+// the biased exponent of the largest: |result| <= 2^(53 + UP).  Down for both signs (~v, also
+// for -0): split_word's rounding of the two last bits then has no bias; truncated negative values got one.
+template <int UP = 6>
 __device__ __forceinline__ long long double_fixed(long long bits, int E) {
   const int hi = (int)(bits >> 32);
   const int e = (hi >> 20) & 0x7ff;
   const unsigned mh = e ? ((unsigned)hi & 0xfffffu) | 0x100000u : 0u;   // subnormals count as zero
-  const unsigned long long m = ((unsigned long long)mh << 32 | (unsigned)bits) << 6;
+  const unsigned long long m = ((unsigned long long)mh << 32 | (unsigned)bits) << UP;
   const int sh = min(E - e, 63);
   const long long v = (long long)(m >> sh);
-  return hi < 0 ? -v : v;
+  return hi < 0 ? ~v : v;
 }
 
 // (-1)^neg a 2^k rounded to nearest, by integer operations; a result in the normal range.
