@@ -1356,8 +1356,8 @@ int pmg_prolong(pmg_hier hh, int level, const double* uc, double* uf, void* stre
   Hier* h = H(hh);
   if (!h || level < 1 || level > h->L || !uc || !uf) return PMG_EINVAL;
   return guarded(h, [&] {
-    const int st = launch_prolong_split(h->dims[level], h->d64[level].at.sp, uc, uf, (cudaStream_t)stream);
-    if (st != PMG_EINVAL) return st;
+    // not the V-cycle's digit-split form, which has one exponent for all values of an element: its
+    // smoothers mix these anyway, a caller of the prolongation alone gets the plain kernel's precision
     return launch_prolong<double>(h->dims[level], h->dims[level - 1], h->J64[level], h->Jhost[level].data(),
                                   uc, uf, (cudaStream_t)stream);
   });

@@ -127,3 +127,23 @@ def test_apply_errors_have_no_sign(P):
     h.apply(h.L, -u, b)
     s = a + b
     assert abs(int((s > 0).sum()) - int((s < 0).sum())) <= 0.1 * u.numel()
+
+
+@pytest.mark.parametrize("P", [4, 8, 16])
+def test_prolongation_keeps_small_values(P):
+    """A face of a fine element depends on that face of the coarse one alone, and values of 1e-9 to
+    1 keep their relative accuracy on the lines they are formed from (1e-13, as the transfers'
+    parity tests; a line's values enter in mirrored pairs)."""
+    from oracle.mg import Hierarchy as OHier
+    from paper_1603_02524_gb300 import Grid, Hierarchy
+    h, oh = Hierarchy(Grid(3, P, [4, 2, 2], GRID, periodic=False)), OHier(3, P, GRID, False)
+    sc, sf = elem_shape(3, (4, 2, 2), P // 2), elem_shape(3, (4, 2, 2), P)
+    c = syn.rng(150).uniform(-1, 1, size=sc)
+    c[..., 1:-1, 1:-1, 1:-1] *= 1e20                           # off the faces
+    c[..., 0] *= 1e-9                                          # two small faces
+    c[..., -1] *= 1e-9
+    out = torch.zeros(int(np.prod(sf)), dtype=torch.float64, device="cuda")
+    h.prolong(h.L, to_dev(c), out)
+    got, ref = from_dev(out, sf), g2e(oh.prolong(h.L, e2g(c, 3)), (4, 2, 2), P)
+    for face in [(..., 0), (..., P), (..., 0, slice(1, P)), (..., P, slice(1, P), slice(1, P))]:
+        assert np.abs(got[face] - ref[face]).max() <= 1e-13 * np.abs(ref[face]).max()
