@@ -328,11 +328,8 @@ __device__ __forceinline__ double coarse_scale(const LevelDims& dm, const Coarse
 // One pass over all lines of an axis, nl lines per CTA staged in shared memory: forward
 // transform (MODE 0), backward (1), or on the last axis forward, scaling by the inverse
 // eigenvalue sums and backward at once (2).  The S tables are read with consecutive outputs
-// in consecutive lanes (forward S, backward its transpose ST).
-//
-// Seven passes took seven launches inside graphs; the fused last axis leaves five (2-D:
-// three), and an fp32 V-cycle's vectors are read and written as they are (two conversion
-// launches fewer).
+// in consecutive lanes (forward S, backward its transpose ST).  Five launches in 3-D, three in
+// 2-D, on the vectors of the V-cycle's own precision; one more for a last axis beyond kCoarseLine.
 template <int MODE, typename TI, typename TO>
 __global__ void __launch_bounds__(128)
 coarse_lines_kernel(LevelDims dm, CoarseFdm c, int axis, int nl, const TI* __restrict__ in, TO* __restrict__ out,
@@ -385,6 +382,36 @@ coarse_lines_kernel(LevelDims dm, CoarseFdm c, int axis, int nl, const TI* __res
   }
 }
 
+// One pass over the lines of a long axis: a CTA forms 128 outputs of a line, whose inputs are
+// staged a chunk at a time, so the length has no limit.  MODE 0, 1 as above; 3: forward and scaling.
+constexpr int kCoarseLine = 2048;         // longest line of coarse_lines_kernel
+template <int MODE, typename TI, typename TO>
+__global__ void __launch_bounds__(128)
+coarse_long_kernel(LevelDims dm, CoarseFdm c, int axis, const TI* __restrict__ in, TO* __restrict__ out, double tol) {
+  constexpr int CHUNK = 1024;
+  __shared__ double a[CHUNK];
+  const int NX = dm.ne[0] * 2, NY = dm.ne[1] * 2, NZ = (dm.dim == 3) ? dm.ne[2] * 2 : 1;
+  const int N = axis == 0 ? NX : axis == 1 ? NY : NZ, n1 = axis == 0 ? NY : NX;
+  const int u = (int)(blockIdx.x % n1), w = (int)(blockIdx.x / n1), o = blockIdx.y * 128 + threadIdx.x;
+  const double* M = MODE == 1 ? (axis == 0 ? c.ST[0] : axis == 1 ? c.ST[1] : c.ST[2])
+                              : (axis == 0 ? c.S[0] : axis == 1 ? c.S[1] : c.S[2]);
+  auto X = [&](int q) { return axis == 0 ? q : u; };
+  auto Y = [&](int q) { return axis == 0 ? u : axis == 1 ? q : w; };
+  auto Z = [&](int q) { return axis == 2 ? q : w; };
+  double s = 0.0;
+  for (int k0 = 0; k0 < N; k0 += CHUNK) {
+    const int nk = min(CHUNK, N - k0);
+    __syncthreads();
+    for (int k = threadIdx.x; k < nk; k += 128) a[k] = (double)in[coarse_off(dm, X(k0 + k), Y(k0 + k), Z(k0 + k))];
+    __syncthreads();
+    if (o < N) {
+#pragma unroll 8
+      for (int k = 0; k < nk; ++k) s = fma(__ldg(M + (size_t)(k0 + k) * N + o), a[k], s);
+    }
+  }
+  if (o < N) out[coarse_off(dm, X(o), Y(o), Z(o))] = (TO)(MODE == 3 ? coarse_scale(dm, c, X(o), Y(o), Z(o), s, tol) : s);
+}
+
 // The whole solve in one CTA, for coarse grids whose passes are shorter than a launch.
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(512)
@@ -432,23 +459,46 @@ int launch_coarse_fdm(const LevelDims& dm, const CoarseFdm& c, const TIO* f, TIO
     coarse_small_kernel<TIO, TIO><<<1, threads, 2 * sizeof(double) * total, s>>>(dm, c, f, u, tol);
     return cudaGetLastError() == cudaSuccess ? PMG_OK : PMG_ECUDA;
   }
-  auto pass = [&](int axis, int mode, auto kernel, auto in, auto out) {
-    const int N = c.N[axis], nl = N < 128 ? 128 / N : 1;
-    const size_t smem = sizeof(double) * (size_t)nl * N * (mode == 2 ? 2 : 1);
+  const int last = dm.dim - 1;
+  int rc = PMG_OK;
+  // mode 0: forward, 1: backward, 2: forward, scaled and backward, 3: forward and scaled
+  auto pass = [&](int axis, auto mode, auto in, auto out) {
+    using TI = std::remove_cv_t<std::remove_pointer_t<decltype(in)>>;
+    using TO = std::remove_pointer_t<decltype(out)>;
+    constexpr int MODE = decltype(mode)::value;
+    if (rc != PMG_OK) return;
+    const int N = c.N[axis];
     const long long lines = total / N;
-    if (!set_smem(kernel, smem)) return (int)PMG_ECUDA;
     count_launch();
-    kernel<<<(unsigned)((lines + nl - 1) / nl), 128, smem, s>>>(dm, c, axis, nl, in, out, tol);
-    return cudaGetLastError() == cudaSuccess ? (int)PMG_OK : (int)PMG_ECUDA;
+    if constexpr (MODE != 2) {
+      if (N > kCoarseLine)
+        coarse_long_kernel<MODE, TI, TO><<<dim3((unsigned)lines, (N + 127) / 128), 128, 0, s>>>(dm, c, axis, in, out, tol);
+    }
+    if constexpr (MODE != 3) {
+      if (N <= kCoarseLine) {
+        const int nl = N < 128 ? 128 / N : 1;
+        const size_t smem = sizeof(double) * (size_t)nl * N * (MODE == 2 ? 2 : 1);
+        coarse_lines_kernel<MODE, TI, TO><<<(unsigned)((lines + nl - 1) / nl), 128, smem, s>>>(dm, c, axis, nl, in, out, tol);
+      }
+    }
+    if (cudaGetLastError() != cudaSuccess) rc = PMG_ECUDA;
   };
-  const bool d3 = dm.dim == 3;
-  double *t0 = c.tmp[0], *t1 = c.tmp[1];
-  int rc = pass(0, 0, coarse_lines_kernel<0, TIO, double>, f, t0);
-  if (rc == PMG_OK && d3) rc = pass(1, 0, coarse_lines_kernel<0, double, double>, (const double*)t0, t1);
-  if (rc == PMG_OK) rc = d3 ? pass(2, 2, coarse_lines_kernel<2, double, double>, (const double*)t1, t0)
-                            : pass(1, 2, coarse_lines_kernel<2, double, double>, (const double*)t0, t1);
-  if (rc == PMG_OK && d3) rc = pass(1, 1, coarse_lines_kernel<1, double, double>, (const double*)t0, t1);
-  if (rc == PMG_OK) rc = pass(0, 1, coarse_lines_kernel<1, double, TIO>, (const double*)t1, u);
+  double* t[2] = {c.tmp[0], c.tmp[1]};
+  int k = 0;
+  pass(0, std::integral_constant<int, 0>{}, f, t[0]);
+  auto next = [&](int axis, auto mode) {
+    pass(axis, mode, (const double*)t[k], t[k ^ 1]);
+    k ^= 1;
+  };
+  if (last == 2) next(1, std::integral_constant<int, 0>{});
+  if (c.N[last] > kCoarseLine) {
+    next(last, std::integral_constant<int, 3>{});
+    next(last, std::integral_constant<int, 1>{});
+  } else {
+    next(last, std::integral_constant<int, 2>{});
+  }
+  if (last == 2) next(1, std::integral_constant<int, 1>{});
+  pass(0, std::integral_constant<int, 1>{}, (const double*)t[k], u);
   return rc;
 }
 template int launch_coarse_fdm<double>(const LevelDims&, const CoarseFdm&, const double*, double*, cudaStream_t);
