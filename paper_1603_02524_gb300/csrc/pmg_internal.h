@@ -213,6 +213,15 @@ struct LevelDims {
 };
 
 // all device allocations of one level, for one scalar type
+// Device memory of one part of a hierarchy.  Small tables share blocks: their values are collected
+// in a host image of the open block and copied together (flush_tables).
+struct DeviceMemory {
+  std::vector<void*> blocks;
+  std::vector<char> image;                 // values of the open block's first bytes
+  char* open = nullptr;
+  size_t cap = 0, flushed = 0;
+};
+
 template <typename T>
 struct LevelDev {
   ApplyTables<T> at{};
@@ -221,7 +230,7 @@ struct LevelDev {
   T* u = nullptr;      // level solution / correction
   T* f = nullptr;      // level right-hand side
   T* r = nullptr;      // residual scratch
-  std::vector<void*> owned;
+  DeviceMemory owned;
 };
 
 struct CoarseFdm {            // exact global fast-diagonalisation solve at P = 1
@@ -285,7 +294,7 @@ struct Hier {
   int* duz = nullptr;              // 1 if the solve's initial u has a nonzero entry
   double* hscal = nullptr;         // pinned host mirror (host_mirror_bytes): control words, results
   double *g_host_stage = nullptr, *u_host_stage = nullptr;   // device buffers for solve_host
-  std::vector<void*> owned;
+  DeviceMemory owned;
   std::string err;
   int nsm = 152;
   // CUDA graph of the MGCG preconditioner (V-cycle r -> z on the fixed work

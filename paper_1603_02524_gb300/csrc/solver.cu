@@ -64,25 +64,51 @@ struct CudaError : std::exception {
   } while (0)
 
 template <typename T>
-T* dev_alloc(std::vector<void*>& owned, size_t count) {
+T* dev_alloc(DeviceMemory& owned, size_t count) {
   void* p = nullptr;
   PMG_CUDA(cudaMalloc(&p, count * sizeof(T) + 16));
-  owned.push_back(p);
+  owned.blocks.push_back(p);
   return static_cast<T*>(p);
 }
 
-template <typename T>
-T* dev_upload(std::vector<void*>& owned, const std::vector<double>& host) {
-  std::vector<T> tmp(host.begin(), host.end());
-  T* d = dev_alloc<T>(owned, tmp.size() ? tmp.size() : 1);
-  if (!tmp.empty()) PMG_CUDA(cudaMemcpy(d, tmp.data(), tmp.size() * sizeof(T), cudaMemcpyHostToDevice));
-  return d;
+void flush_tables(DeviceMemory& m) {
+  if (m.image.size() > m.flushed)
+    PMG_CUDA(cudaMemcpy(m.open + m.flushed, m.image.data() + m.flushed, m.image.size() - m.flushed, cudaMemcpyHostToDevice));
+  m.flushed = m.image.size();
 }
 
-int* dev_upload_int(std::vector<void*>& owned, const std::vector<int>& host) {
-  int* d = dev_alloc<int>(owned, host.size() ? host.size() : 1);
-  if (!host.empty()) PMG_CUDA(cudaMemcpy(d, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice));
-  return d;
+// Device copy of a table, valid once flush_tables has run.  A hierarchy has hundreds of them, most of a
+// few kB; an allocation and a synchronous copy for each took most of a small one's set-up.
+void* upload_bytes(DeviceMemory& m, const void* src, size_t bytes) {
+  constexpr size_t kBlock = 1u << 18;
+  const size_t room = (bytes + 16 + 255) / 256 * 256;
+  if (room > kBlock / 4) {
+    char* p = dev_alloc<char>(m, bytes);
+    PMG_CUDA(cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice));
+    return p;
+  }
+  if (m.image.size() + room > m.cap) {
+    flush_tables(m);
+    m.open = dev_alloc<char>(m, kBlock);
+    m.cap = kBlock;
+    m.flushed = 0;
+    m.image.clear();
+    m.image.reserve(kBlock);
+  }
+  const size_t at = m.image.size();
+  m.image.resize(at + room);
+  if (bytes) std::memcpy(m.image.data() + at, src, bytes);
+  return m.open + at;
+}
+
+template <typename T>
+T* dev_upload(DeviceMemory& owned, const std::vector<double>& host) {
+  std::vector<T> tmp(host.begin(), host.end());
+  return static_cast<T*>(upload_bytes(owned, tmp.data(), tmp.size() * sizeof(T)));
+}
+
+int* dev_upload_int(DeviceMemory& owned, const std::vector<int>& host) {
+  return static_cast<int*>(upload_bytes(owned, host.data(), host.size() * sizeof(int)));
 }
 
 // per-level smoother parameters (0 selects the default)
@@ -95,7 +121,7 @@ double level_tau(const pmg_options& o, int l) {
 
 // trivial third axis of a 2-D patch family
 template <typename T>
-FdmAxis<T> trivial_axis(std::vector<void*>& owned) {
+FdmAxis<T> trivial_axis(DeviceMemory& owned) {
   FdmAxis<T> ax{};
   ax.n = 1;
   ax.count = 1;
@@ -127,7 +153,7 @@ double round_to_tf32(double x) {
 // scale: omega for the first patch-buffer axis (folds the damping into W), 1 otherwise;
 // tf32: tables rounded to tf32 for the tensor-core patch kernel
 template <typename T>
-FdmAxis<T> upload_axis(std::vector<void*>& owned, const AxisTables& t, const Axis1DHost& a, int phys,
+FdmAxis<T> upload_axis(DeviceMemory& owned, const AxisTables& t, const Axis1DHost& a, int phys,
                        double scale, bool tf32 = false) {
   FdmAxis<T> ax{};
   ax.n = t.n;
@@ -170,15 +196,13 @@ FdmAxis<T> upload_axis(std::vector<void*>& owned, const AxisTables& t, const Axi
   return ax;
 }
 
-uint4* upload_frag(std::vector<void*>& owned, const std::vector<uint32_t>& f) {
-  uint32_t* d = dev_alloc<uint32_t>(owned, f.size());
-  PMG_CUDA(cudaMemcpy(d, f.data(), f.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
-  return reinterpret_cast<uint4*>(d);
+uint4* upload_frag(DeviceMemory& owned, const std::vector<uint32_t>& f) {
+  return static_cast<uint4*>(upload_bytes(owned, f.data(), f.size() * sizeof(uint32_t)));
 }
 
 // Digit fragments of the operator of level l and of its transfers (apply_split.cuh): 3-D,
 // orders 4, 8 and 16; one table per distinct element of an axis.
-void attach_split_apply(Hier& h, int l, SplitApply& sp, std::vector<void*>& own) {
+void attach_split_apply(Hier& h, int l, SplitApply& sp, DeviceMemory& own) {
   const LevelDims& dm = h.dims[l];
   if (dm.dim != 3 || (dm.NP != 5 && dm.NP != 9 && dm.NP != 17)) return;
   bool ok = true;
@@ -237,7 +261,7 @@ void attach_split_apply(Hier& h, int l, SplitApply& sp, std::vector<void*>& own)
 
 // operator-apply tables of level l in arithmetic T
 template <typename T>
-ApplyTables<T> build_apply_tables(Hier& h, int l, std::vector<void*>& own) {
+ApplyTables<T> build_apply_tables(Hier& h, int l, DeviceMemory& own) {
   const LevelDims& dm = h.dims[l];
   auto& ax = h.axes[l];
   ApplyTables<T> at{};
@@ -278,7 +302,7 @@ size_t patch_smem_bytes(int n0, int n1, int n2) {
 }
 
 template <typename T>
-void attach_scratch(Hier& h, FdmFamily<T>& fam, std::vector<void*>& own) {
+void attach_scratch(Hier& h, FdmFamily<T>& fam, DeviceMemory& own) {
   const int n0 = fam.ax[0].n, n1 = fam.ax[1].n, n2 = fam.ax[2].n;
   if (patch_smem_bytes<T>(n0, n1, n2) <= 227 * 1024) return;
   fam.scratch_stride = ((long long)(n0 * n1 + 7) / 8 * 8 * n2 + 31) / 32 * 32;   // planes of whole sectors (fp32)
@@ -298,7 +322,7 @@ void attach_scratch(Hier& h, FdmFamily<T>& fam, std::vector<void*>& own) {
 // table is small and the patch kernel replaces a Newton reciprocal per node by one
 // load.  Skipped when the combinations would take more than 32 MB.
 template <typename T>
-void attach_inverse_table(FdmFamily<T>& fam, const AxisTables* const (&tab)[3], std::vector<void*>& own) {
+void attach_inverse_table(FdmFamily<T>& fam, const AxisTables* const (&tab)[3], DeviceMemory& own) {
   if (sizeof(T) != 8 || fam.tc) return;
   std::vector<int> uid[3];
   std::vector<std::vector<double>> rep[3];
@@ -348,7 +372,7 @@ void attach_inverse_table(FdmFamily<T>& fam, const AxisTables* const (&tab)[3], 
 // exactness bound.
 template <typename T>
 void attach_split(FdmFamily<T>& fam, const LevelDims& dm, const AxisTables* const (&tab)[3], double omega,
-                  std::vector<void*>& own) {
+                  DeviceMemory& own) {
   constexpr bool fp64 = sizeof(T) == 8;
   bool ok = true;
   long long nodes = 1;
@@ -428,9 +452,7 @@ void attach_split(FdmFamily<T>& fam, const LevelDims& dm, const AxisTables* cons
                                         : (long long)(G / npp) * es[ax.phys] + (G % npp) * ns[ax.phys];
       }
     }
-    long long* d = dev_alloc<long long>(own, off.size());
-    PMG_CUDA(cudaMemcpy(d, off.data(), off.size() * sizeof(long long), cudaMemcpyHostToDevice));
-    ax.goff = d;
+    ax.goff = static_cast<const long long*>(upload_bytes(own, off.data(), off.size() * sizeof(long long)));
   }
   fam.split = ok ? 1 : 0;
 }
@@ -1005,13 +1027,13 @@ struct Batch {
   SolveResult* hres = nullptr;     // pinned host [total segments]
   std::vector<int> off;            // first segment of solve i
   std::vector<unsigned long long> fixed, per_iter;
-  std::vector<void*> owned;
+  DeviceMemory owned;
   std::string err;
 };
 
 void free_batch(Batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
-  for (void* p : b->owned) cudaFree(p);
+  for (void* p : b->owned.blocks) cudaFree(p);
   if (b->hres) cudaFreeHost(b->hres);
   delete b;
 }
@@ -1037,10 +1059,10 @@ int guarded(Hier* h, F&& fn) {
 
 void free_all(Hier* h) {
   for (int l = 0; l < kMaxLevels; ++l) {
-    for (void* p : h->d64[l].owned) cudaFree(p);
-    for (void* p : h->d32[l].owned) cudaFree(p);
+    for (void* p : h->d64[l].owned.blocks) cudaFree(p);
+    for (void* p : h->d32[l].owned.blocks) cudaFree(p);
   }
-  for (void* p : h->owned) cudaFree(p);
+  for (void* p : h->owned.blocks) cudaFree(p);
   if (h->hscal) cudaFreeHost(h->hscal);
   if (h->pc_exec) cudaGraphExecDestroy(h->pc_exec);
   if (h->sv_exec) cudaGraphExecDestroy(h->sv_exec);
@@ -1256,6 +1278,11 @@ int pmg_hierarchy_build(pmg_grid g, const pmg_options* opt, pmg_hier* out) {
       h->d32[l].ea.status = h->dstatus;
       for (int q = 0; q < 3; ++q) h->d32[l].fa[q].status = h->dstatus;
     }
+    for (int l = 0; l <= L; ++l) {
+      flush_tables(h->d64[l].owned);
+      flush_tables(h->d32[l].owned);
+    }
+    flush_tables(h->owned);
     PMG_CUDA(cudaDeviceSynchronize());
     return PMG_OK;
   });
