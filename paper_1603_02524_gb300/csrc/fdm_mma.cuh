@@ -36,8 +36,7 @@ struct MmaShape {
   static constexpr size_t LAM = ROW + 8 * (size_t)(NB * NC);
   static constexpr size_t BUF = LAM + 4 * (size_t)NOFF;
   static constexpr size_t BYTES = BUF + 4 * (size_t)NN;
-  static constexpr int THREADS = NC == 1 ? ((NA > NB ? NA : NB) + 7) / 8 * 32
-                                         : NN > 14000 ? 512 : NN > 6000 ? 256 : NN > 300 ? 128 : 64;
+  static constexpr int THREADS = patch_threads(NA, NB, NC);
   static constexpr int MINB = (NA > 16 || NB > 16 ? 768 : 1024) / THREADS;   // 80 or 64 registers per thread
 };
 

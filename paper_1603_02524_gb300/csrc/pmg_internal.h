@@ -157,6 +157,11 @@ __host__ __device__ __forceinline__ int patch_start(const FdmAxis<T>& ax, int p,
 
 // offset contribution of a patch node outside the domain (any sum with one is negative)
 constexpr long long kInvalidOffset = -(1LL << 60);
+// CTA size of the tensor-core patch kernels on patches of na x nb x nc nodes, the largest that they
+// take (nc = 1: 2-D, one tile of eight lines per warp and pass).
+__host__ __device__ constexpr int patch_threads(int na, int nb, int nc) {
+  return nc == 1 ? ((na > nb ? na : nb) + 7) / 8 * 32 : na * nb * nc > 14000 ? 512 : na * nb * nc > 6000 ? 256 : 128;
+}
 // Largest CTA any patch-kernel launch may use (the autotuner's candidates stay
 // within it; it caps registers at 128 per thread).
 constexpr int kFdmMaxThreads = 512;

@@ -898,18 +898,19 @@ int solve_graph_run(Hier& h, pmg_stats* st, cudaStream_t s) {
 // process, so many hierarchies of one shape tune once.
 // ---------------------------------------------------------------------------
 std::mutex g_tune_mu;
-std::map<std::array<int, 6>, int> g_tune_cache;
+std::map<std::array<int, 7>, int> g_tune_cache;   // CTA size + 1000 (variant + 1)
 
 template <typename T>
 int tune_family(Hier& h, int l, FdmFamily<T>& fam, LevelDev<T>& d, cudaStream_t s) {
+  if (sizeof(T) == 4 && fam.split && fam.ax[1].n > 32) return 0;      // the slab kernels: one CTA size
   int lg = 0;
   while ((1 << (lg + 1)) <= fam.count_total) ++lg;
-  const std::array<int, 6> key = {(int)sizeof(T), fam.ax[0].n, fam.ax[1].n, fam.ax[2].n, fam.tc, lg};
+  const std::array<int, 7> key = {(int)sizeof(T), fam.ax[0].n, fam.ax[1].n, fam.ax[2].n, fam.tc, fam.split, lg};
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
-      fam.variant = it->second / 1000;
+      fam.variant = it->second / 1000 - 1;
       return fam.threads = it->second % 1000;
     }
   }
@@ -923,6 +924,8 @@ int tune_family(Hier& h, int l, FdmFamily<T>& fam, LevelDev<T>& d, cudaStream_t 
   const bool tc5 = sizeof(T) == 4 && fam.tc == 2 && dm.dim == 3;
   const int* cand = tc5 ? cand_tc : cand_simt;
   const int ncand = tc5 ? 4 : 10;
+  // the tensor-core kernels take any size up to their own: smaller ones, and that one
+  const int top = fam.split ? patch_threads(fam.ax[0].n, fam.ax[1].n, fam.ax[2].n) : kFdmMaxThreads;
   cudaEvent_t e0, e1;
   PMG_CUDA(cudaEventCreate(&e0));
   PMG_CUDA(cudaEventCreate(&e1));
@@ -934,8 +937,8 @@ int tune_family(Hier& h, int l, FdmFamily<T>& fam, LevelDev<T>& d, cudaStream_t 
   try {
     for (int v = 0; v < nvar; ++v) {
       for (int ci = 0; ci < ncand; ++ci) {
-        const int c = cand[ci];
-        if (c > kFdmMaxThreads) continue;
+        const int c = cand[ci] < top ? cand[ci] : top;
+        if (ci > 0 && cand[ci - 1] >= top) break;
         fam.threads = c;
         fam.variant = nvar == 2 ? v : -1;
         PMG_CHECK(launch_fdm<T>(dm, fam, d.f, d.u, s));            // warm-up
@@ -964,7 +967,7 @@ int tune_family(Hier& h, int l, FdmFamily<T>& fam, LevelDev<T>& d, cudaStream_t 
   fam.threads = best;
   fam.variant = best_v;
   std::lock_guard<std::mutex> lock(g_tune_mu);
-  g_tune_cache[key] = best + 1000 * (best_v < 0 ? 0 : best_v);
+  g_tune_cache[key] = best + 1000 * (best_v + 1);
   return best;
 }
 
