@@ -69,12 +69,18 @@ enum { PMG_WEIGHT_UNWEIGHTED = 0, PMG_WEIGHT_ARITHMETIC = 1, PMG_WEIGHT_CUBIC = 
  * residuals, transfers) inside the FP64 flexible CG (spec extension), with
  * the patch transforms on the SIMT cores (MIXED) or on the tensor cores (MIXED_TC:
  * mma.sync TF32 with the 3xTF32 split, i.e. fp32-level products and fp32
- * accumulation; 3-D patches of at most 32 nodes per axis, others stay SIMT). */
+ * accumulation; 3-D patches of at most 32 nodes per axis).  MIXED, and the patches
+ * that the other two leave out, use the SIMT cores or three-term bf16 products of
+ * fp32 accuracy on the tensor cores, by the patch size.
+ * FP64 patch solves, operator applies and the V-cycle's transfers (3-D, P = 4, 8, 16) run on
+ * the tensor cores as exact products of integer digits.  A patch solve carries
+ * 59 bits below the largest residual of its patch, an apply FP64 precision
+ * relative to the lines through a node. */
 enum { PMG_PREC_FP64 = 0, PMG_PREC_MIXED = 1, PMG_PREC_MIXED_TC = 2, PMG_PREC_MIXED_TF32 = 3 };
 /* PMG_PREC_MIXED_TF32: one TF32 product per multiply-add (10-bit operand
  * mantissas, fp32 accumulation), the patch line passes as tcgen05 MMAs with the
  * operands in shared memory and the accumulators in tensor memory (3-D patches
- * of at most 32 nodes per axis; others stay SIMT): a lower-precision
+ * of 13^3 to 32^3 nodes; others as MIXED): a lower-precision
  * preconditioner whose effect on the iteration count the flexible CG absorbs. */
 /* Preconditioner of the CG iteration (Algorithm 2). */
 enum { PMG_PC_VCYCLE = 0, PMG_PC_NONE = 1 };
@@ -82,7 +88,9 @@ enum { PMG_PC_VCYCLE = 0, PMG_PC_NONE = 1 };
  * emulated FP64 in double-float (DF: each value the sum of two fp32 words,
  * about 48 significant bits, products split exactly by FMA and sums by TwoSum)
  * on the FP32 pipes, which on GB300 issue ~60x the FP64 rate.  DF needs the
- * vector and operator magnitudes within fp32's exponent range (~1e-30..1e30). */
+ * vector and operator magnitudes within fp32's exponent range (~1e-30..1e30).
+ * On 3-D grids of P = 16 DF runs the FP64 apply, which is as fast there (its
+ * contractions run on the tensor cores as exact digit products). */
 enum { PMG_OUTER_FP64 = 0, PMG_OUTER_DF = 1 };
 
 typedef struct {

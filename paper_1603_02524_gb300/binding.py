@@ -122,7 +122,7 @@ def options(smoother="EA", overlap="l", weighting="quintic", ns=(1, 1), variable
             preconditioner="vcycle", outer_apply="fp64", nrhs=1) -> PmgOptions:
     """omega_level / tau_level: optional per-level sequences (index = level, 0 = default);
     preconditioner "vcycle" (Algorithm 2) or "none" (plain CG); outer_apply "fp64" or "df"
-    (the CG's operator apply in double-float on the FP32 pipes)."""
+    (the CG's operator apply in double-float on the FP32 pipes; FP64 too on 3-D grids of P = 16)."""
     o = PmgOptions()
     load().pmg_options_default(ctypes.byref(o))
     o.smoother = SMOOTHER[smoother]

@@ -696,14 +696,19 @@ void precondition_graph(Hier& h, cudaStream_t s) {
   if (h.pc_state == 0) h.pc_launches = g_launches.load() - c0;
 }
 
+// Whether the outer apply runs in double-float.  3-D P = 16: the digit-split FP64 apply takes as long
+// (16^3 elements: both 0.74 ms) and has all of FP64's precision and range; at P = 8 double-float
+// takes 0.098 ms against 0.137.
+bool outer_df(const Hier& h) {
+  const LevelDims& dm = h.dims[h.L];
+  return h.opt.outer_apply == PMG_OUTER_DF && !(dm.dim == 3 && dm.NP == 17);
+}
 // The outer CG's operator apply on the finest level: v = A u, or v = f - A u
 // (f non-null); FP64, or double-float on the FP32 pipes (outer_apply option).
 void outer_apply(Hier& h, const double* u, const double* f, double* v, cudaStream_t s,
                  const int* unz = nullptr) {
   const LevelDims& dm = h.dims[h.L];
-  // P = 16: the digit-split FP64 apply is the faster one (16^3 elements: 0.74 -> 0.70 ms), and
-  // the more accurate; at P = 8 double-float takes 0.105 ms against 0.128
-  if (h.opt.outer_apply == PMG_OUTER_DF && !(dm.NP == 17 && h.d64[h.L].at.sp.ok)) {
+  if (outer_df(h)) {
     PMG_CHECK(launch_apply_df(dm, h.at_df, u, f, v, s, unz));
   } else {
     PMG_CHECK(launch_apply<double>(dm, h.d64[h.L].at, u, f, v, s, unz));
@@ -1238,7 +1243,7 @@ int pmg_hierarchy_build(pmg_grid g, const pmg_options* opt, pmg_hier* out) {
       }
     }
     h->has32 = o.precision != PMG_PREC_FP64;
-    if (o.outer_apply == PMG_OUTER_DF) h->at_df = build_apply_tables<dfloat>(*h, L, h->owned);
+    if (outer_df(*h)) h->at_df = build_apply_tables<dfloat>(*h, L, h->owned);
     // exact coarse solve tables (global 1-D eigen-pairs at P = 1)
     CoarseFdm& c = h->coarse;
     c.lam_max = 0.0;
