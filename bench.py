@@ -70,7 +70,7 @@ def patch_kernel(prec, dim, na, nn, peaks):
         return ("fdm_kernel_tc", TF32_PEAK_GFLOPS, "dense tf32 tensor peak = measured bf16 burst peak x 1/2; flops are "
                 "the line passes' multiply-adds x 2 (tables unfolded)")
     if prec == "fp64" and na <= 32 and nodes >= (300 if dim == 3 else 20):
-        return ("fdm_kernel_split", tensor / 21, "measured bf16 burst peak / 21: an FP64 multiply-add takes 21 fp16 "
+        return ("fdm_kernel_split", tensor / 26, "measured bf16 burst peak / 26: an FP64 multiply-add takes 26 fp16 "
                 "products of its operands' digits on the tensor cores")
     if prec in ("mixed", "mixed_tf32") and (na <= 32 or dim == 3 and nodes > 58000) and \
             nodes >= (20 if dim == 2 else 1000 if na == nn else 600):

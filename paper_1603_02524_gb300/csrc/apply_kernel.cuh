@@ -162,9 +162,9 @@ static bool set_smem(K fn, size_t bytes) {
 // (sum_k D_{P,k} u_k^{m-1}, sum_k D_{0,k} u_k^{m+1}).  The axes accumulate in
 // shared memory; the last one multiplies by the masses and writes v from registers.
 //
-// What bounds it (fp32, 3-D): the load unit (68 % busy at P = 16, 53 % at P = 8) and the
-// latency of the neighbour reads, which used to precede each axis pass (long-scoreboard
-// stalls 13.6 of 21 cycles per instruction).  Now the ends of all axes are read at the start,
+// What bounds it (fp32, 3-D): the load unit (72 % busy at P = 8) and the latency of the
+// neighbour reads, which used to precede each axis pass (long-scoreboard stalls 13.6 of 21
+// cycles per instruction, load unit 53 %).  Now the ends of all axes are read at the start,
 // the x neighbours through shared memory (apply_staged), and the last pass needs no sweep of
 // its own.  fp32 residuals: P = 8 at 8192 elements 76 -> 54 us, P = 16 at 4096 elements
 // 240 -> 200, its fused restriction 257 -> 213, P = 2 at 8192 12.2 -> 9.3; FP64 2-D solves

@@ -8,7 +8,6 @@
 // four multiply-adds, and that traffic was their bound.  Here the table fragments stay in
 // registers for all the tiles of a pass.
 //
-//
 // Precision: the tensor core rounds its sums toward zero; the tables carry the mean of that
 // (bf16_fragments), and each output is rounded once at full scale (inputs beyond 16 go to a
 // second accumulator).  A sweep's error against FP64 is 7-9e-8 of its norm, the SIMT passes'

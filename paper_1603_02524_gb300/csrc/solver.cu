@@ -474,8 +474,8 @@ void build_level_dev(Hier& h, int l, LevelDev<T>& dev, const std::vector<AxisTab
                : 0;
   if (dm.NP > 32) tc = 0;                 // P = 32 patches: the slab kernel (fdm_mma.cuh)
   if (tc == 2) {
-    // the tcgen05 kernel pays a fixed latency per line pass; small patches stay on
-    // the SIMT kernel (folded tables), which is faster there
+    // the tcgen05 kernel pays a fixed latency per line pass; small patches stay on the kernels
+    // of fp32 accuracy (bf16-term MMA or SIMT, attach_split), which are faster there
     const long long nn = (long long)(h.opt.smoother == PMG_SMOOTHER_EA ? ec[0].n : fc[0].n) * ec[1].n * ec[2].n;
     if (nn < kTcMinPatchNodes) tc = 0;
   }
